@@ -283,6 +283,14 @@ Region grow(const Region& r, int k, int nx, int ny, int nz) {
     return o;
 }
 
+// Where the phase-by-phase kernels stream for a box R: the collision on R reads
+// colour fractions on R grown by one ring. A box that stands on the substrate
+// reads them on the ghost plane z = -1 too, each a mean over the densities of
+// plane 0 one ring further out (Eq. 18), so that box streams two rings. (With
+// one, a ghost value at the box's edge mixed in a density that no kernel had
+// written in the step.)
+Region stream_region(const Region& R, int nx, int ny, int nz) { return grow(R, R.z0 == 0 ? 2 : 1, nx, ny, nz); }
+
 // box around the nozzle wall at steps n0 and n0 + 1 (the step that n0 + 1
 // completes). Sites of margin around the wall: a bulk site's own pull and the
 // pulls of its neighbours (for their colour fractions) must see no wall node,
@@ -385,7 +393,8 @@ lbm_status do_steps(lbm_handle* h, int nsteps) {
                 if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->fork, 0);
                 if (e != cudaSuccess) return cuda_check(h, e, "fork");
                 if ((st = mark(h, 1, false, 0, h->side)) != LBM_OK) return st;
-                launched += launch_plain<VS, real, S>(p, box, grow(box, 1, nx, ny, nz), h->side);
+                launched += launch_plain<VS, real, S>(p, box, grow(box, 1, nx, ny, nz),
+                                                      stream_region(box, nx, ny, nz), h->side);
                 if ((st = mark(h, 1, true, box_sites, h->side)) != LBM_OK) return st;
             }
             if ((st = mark(h, 0, false, 0, h->stream)) != LBM_OK) return st;
@@ -399,7 +408,7 @@ lbm_status do_steps(lbm_handle* h, int nsteps) {
         } else {
             const Region R = full_region(h);
             if ((st = mark(h, 1, false, 0, h->stream)) != LBM_OK) return st;
-            launched += launch_plain<VS, real, S>(p, R, R, h->stream);
+            launched += launch_plain<VS, real, S>(p, R, R, R, h->stream);
             if ((st = mark(h, 1, true, h->N, h->stream)) != LBM_OK) return st;
         }
         h->launches += launched;
@@ -913,7 +922,7 @@ lbm_status noalloc_step(lbm_handle* tmp, long long step, const void* f_in, void*
     p.geo = geo;
     launch_prev_from_f<VS, real>(p, rho_prev, u_prev, st);
     const Region R = full_region(tmp);
-    launch_plain<VS, real, real>(p, R, R, st, true);
+    launch_plain<VS, real, real>(p, R, R, R, st, true);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(nullptr, LBM_ECUDA, "lbm_step_noalloc: launch: %s", cudaGetErrorString(e));
     if (!diag) return LBM_OK;
@@ -1117,8 +1126,8 @@ lbm_status batch_plan(lbm_batch* b, int variant, const std::vector<int>& zc) {
     return LBM_OK;
 }
 
-// grid of the batched box kernels: the columns of the nozzle flags (the box
-// grown by three rings, so that the box can move for a while before the
+// grid of the batched box kernels: the columns of the nozzle flags (two rings
+// around the streamed ones, so that the box can move for a while before the
 // captured graph needs a larger grid) and the planes of the colour phase
 void box_grid(const Region& Rg, const Region& R1g, unsigned* gx, unsigned* gy) {
     const long long cols = (long long)Rg.wx * Rg.wy;
@@ -1198,10 +1207,11 @@ lbm_status batch_steps(lbm_batch* b, int nsteps) {
                 if (box.wx > 0) {
                     const int nx = h->cfg.nx, ny = h->cfg.ny, nz = h->cfg.nz;
                     q.R1 = grow(box, 1, nx, ny, nz);
+                    q.Rs = stream_region(box, nx, ny, nz);
                     q.R1g = q.R1;
                     if (q.R1g.z0 <= 0) q.R1g.z0 = -1;
                     if (q.R1g.z1 >= nz) q.R1g.z1 = nz + 1;
-                    q.Rg = grow(q.R1, 2, nx, ny, nz);
+                    q.Rg = grow(q.Rs, 2, nx, ny, nz);
                     box_grid(q.Rg, q.R1g, &gx, &gy);
                 }
             }

@@ -32,8 +32,8 @@ __host__ __device__ inline int chunk_begin(int nz, int n, int k, bool guided) {
 }
 
 // Phase-by-phase step over region R (all sites, or the nozzle box):
-//   0. per-column nozzle flags over R grown by three rings (nozzle runs)
-//   1. stream + densities on R grown by one ring, moments and ledger of R
+//   0. per-column nozzle flags over Rs grown by two rings (nozzle runs)
+//   1. stream + densities on Rs (see stream_region), moments and ledger of R
 //   2. created nodes on R grown by one ring (nozzle runs)
 //   3. colour fractions on R grown by one ring, from the fictitious densities on wall nodes and ghost planes
 //   4. collision on R
@@ -41,7 +41,8 @@ __host__ __device__ inline int chunk_begin(int nz, int n, int k, bool guided) {
 // Returns the number of kernels launched.
 // S is the stored population type (see Stored).
 template <class VS, typename real, typename S>
-int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, cudaStream_t st, bool flags_done = false);
+int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, const Region& Rs, cudaStream_t st,
+                 bool flags_done = false);
 
 // Fused bulk step over every site outside p.box (D3Q19, substrate + open top).
 template <typename real, typename S>
@@ -76,7 +77,7 @@ inline int fused_ctas_per_sm(bool fp64) { return fp64 ? 1 : 3; }
 template <typename real>
 struct BoxArgs {
     StepArgs<real> p;
-    Region R, R1, R1g, Rg;  // Rg: the columns of the nozzle flags (R1 and two more rings)
+    Region R, R1, Rs, R1g, Rg;  // Rg: the columns of the nozzle flags (Rs and two more rings)
 };
 template <class VS, typename real, typename S>
 int launch_plain_batch(const BoxArgs<real>* t, int n, unsigned gx, unsigned gy, int unit, cudaStream_t st);

@@ -78,14 +78,14 @@ __global__ void __launch_bounds__(kThreads) k_geo_b(const BoxArgs<real>* __restr
     geo_body(b.p, b.Rg);
 }
 
-// the columns the boundary kernels query around region R1: two more rings
-// (neighbours, and the wall-density extrapolation two links out)
-__host__ __device__ inline Region geo_region(const Region& R1, int nx, int ny) {
-    Region g = R1;
-    if (R1.wx + 4 >= nx) { g.x0 = 0; g.wx = nx; }
-    else { g.x0 = R1.x0 - 2 < 0 ? R1.x0 - 2 + nx : R1.x0 - 2; g.wx = R1.wx + 4; }
-    if (R1.wy + 4 >= ny) { g.y0 = 0; g.wy = ny; }
-    else { g.y0 = R1.y0 - 2 < 0 ? R1.y0 - 2 + ny : R1.y0 - 2; g.wy = R1.wy + 4; }
+// the columns the boundary kernels query around the streamed region Rs: two
+// more rings (neighbours, and the wall-density extrapolation two links out)
+__host__ __device__ inline Region geo_region(const Region& Rs, int nx, int ny) {
+    Region g = Rs;
+    if (Rs.wx + 4 >= nx) { g.x0 = 0; g.wx = nx; }
+    else { g.x0 = Rs.x0 - 2 < 0 ? Rs.x0 - 2 + nx : Rs.x0 - 2; g.wx = Rs.wx + 4; }
+    if (Rs.wy + 4 >= ny) { g.y0 = 0; g.wy = ny; }
+    else { g.y0 = Rs.y0 - 2 < 0 ? Rs.y0 - 2 + ny : Rs.y0 - 2; g.wy = Rs.wy + 4; }
     g.z0 = 0;
     g.z1 = 1;
     return g;
@@ -112,13 +112,13 @@ __device__ __forceinline__ void post_put(const StepArgs<real>& p, long long s, c
     }
 }
 
-// 1. stream + densities (post-streaming) of every fluid node of step n-1 in R1
+// 1. stream + densities (post-streaming) of every fluid node of step n-1 in Rs
 template <class VS, typename real, typename S>
-__device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, const Region& R1, const Region& R) {
+__device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, const Region& Rs, const Region& R) {
     const long long comp = p.N + 2 * p.plane;
     double bc0 = 0, bc1 = 0, de0 = 0, de1 = 0;
     int x, y, z;
-    if (region_site(R1, p.nx, p.ny, &x, &y, &z) && !solid_at(p, x, y, z, 0)) {
+    if (region_site(Rs, p.nx, p.ny, &x, &y, &z) && !solid_at(p, x, y, z, 0)) {
         real f[2][VS::Q];
         real bc[2] = {real(0), real(0)};
         pull_general<VS, S>(p, x, y, z, f, bc);
@@ -148,8 +148,8 @@ __device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, con
 }
 
 template <class VS, typename real, typename S>
-__global__ void __launch_bounds__(kThreads, 2) k_stream_density(StepArgs<real> p, Region R1, Region R) {
-    stream_density_body<VS, real, S>(p, R1, R);
+__global__ void __launch_bounds__(kThreads, 2) k_stream_density(StepArgs<real> p, Region Rs, Region R) {
+    stream_density_body<VS, real, S>(p, Rs, R);
 }
 
 // The same with four threads to a site, one warp of the block for every fourth
@@ -159,15 +159,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_stream_density(StepArgs<real> p
 // Alone it takes as long (25 us in the box of 128x64x64), but its blocks fit
 // beside the bulk kernel's: 20 steps of that run 1.72 -> 1.54 ms.
 template <class VS, typename real, typename S>
-__device__ __forceinline__ void stream_density_split_body(const StepArgs<real>& p, const Region& R1, const Region& R) {
+__device__ __forceinline__ void stream_density_split_body(const StepArgs<real>& p, const Region& Rs, const Region& R) {
     constexpr int Q = VS::Q, NK = (Q + 3) / 4;
     __shared__ real sf[2 * Q][32];
     const long long comp = p.N + 2 * p.plane;
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int t = blockIdx.x * 32 + lane;
-    bool site = t < R1.wx * R1.wy && (int)blockIdx.y < R1.z1 - R1.z0;
-    const int j = t / R1.wx;
-    const int x = wrapn(R1.x0 + t - j * R1.wx, p.nx), y = wrapn(R1.y0 + j, p.ny), z = R1.z0 + (int)blockIdx.y;
+    bool site = t < Rs.wx * Rs.wy && (int)blockIdx.y < Rs.z1 - Rs.z0;
+    const int j = t / Rs.wx;
+    const int x = wrapn(Rs.x0 + t - j * Rs.wx, p.nx), y = wrapn(Rs.y0 + j, p.ny), z = Rs.z0 + (int)blockIdx.y;
     site = site && !solid_at(p, x, y, z, 0);
     const bool inside = site && in_region(R, x, y, z, p.nx, p.ny);
     double bc0 = 0, bc1 = 0;
@@ -218,15 +218,15 @@ __device__ __forceinline__ void stream_density_split_body(const StepArgs<real>& 
 }
 
 template <class VS, typename real, typename S>
-__global__ void __launch_bounds__(kThreads) k_stream_density_split(StepArgs<real> p, Region R1, Region R) {
-    stream_density_split_body<VS, real, S>(p, R1, R);
+__global__ void __launch_bounds__(kThreads) k_stream_density_split(StepArgs<real> p, Region Rs, Region R) {
+    stream_density_split_body<VS, real, S>(p, Rs, R);
 }
 
 template <class VS, typename real, typename S>
 __global__ void __launch_bounds__(kThreads) k_stream_density_split_b(const BoxArgs<real>* __restrict__ t) {
     const BoxArgs<real>& b = t[blockIdx.z];
     if (b.R.wx == 0) return;  // no box for this lattice
-    stream_density_split_body<VS, real, S>(b.p, b.R1, b.R);
+    stream_density_split_body<VS, real, S>(b.p, b.Rs, b.R);
 }
 
 // 2. nodes the nozzle uncovered: mean density of the neighbours that are fluid
@@ -669,21 +669,22 @@ inline bool split_stream(long long sites, bool state) {
 }
 
 template <class VS, typename real, typename S>
-int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, cudaStream_t st, bool flags_done) {
+int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, const Region& Rs, cudaStream_t st,
+                 bool flags_done) {
     if (region_sites(R) == 0) return 0;
     int n = 0;
     if (p.nozzle && !flags_done) {
-        const Region G = geo_region(R1, p.nx, p.ny);
+        const Region G = geo_region(Rs, p.nx, p.ny);
         k_geo<real><<<geo_grid(G), kThreads, 0, st>>>(p, G);
         n = 1;
     }
-    if (split_stream(region_sites(R1), std::is_same<S, Mom>::value)) {
-        const long long cols = (long long)R1.wx * R1.wy;
+    if (split_stream(region_sites(Rs), std::is_same<S, Mom>::value)) {
+        const long long cols = (long long)Rs.wx * Rs.wy;
         k_stream_density_split<VS, real, S>
-            <<<dim3((unsigned)((cols + 31) / 32), (unsigned)(R1.z1 - R1.z0)), kThreads, 0, st>>>(p, R1, R);
+            <<<dim3((unsigned)((cols + 31) / 32), (unsigned)(Rs.z1 - Rs.z0)), kThreads, 0, st>>>(p, Rs, R);
     } else {
         if constexpr (!std::is_same<S, Mom>::value)
-            k_stream_density<VS, real, S><<<region_grid(R1), kThreads, 0, st>>>(p, R1, R);
+            k_stream_density<VS, real, S><<<region_grid(Rs), kThreads, 0, st>>>(p, Rs, R);
     }
     if (p.nozzle) {
         k_created<VS, real, S><<<region_grid(R1), kThreads, 0, st>>>(p, R1, R);
@@ -733,23 +734,23 @@ int launch_init(const StepArgs<real>& p, int staged, int have_u, cudaStream_t st
     return 1 + n;
 }
 
-template int launch_plain<D3Q19, float, float>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D3Q19, float, float>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D3Q19, float, float>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D3Q19, float, Mom>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D3Q19, float, Mom>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D3Q19, float, Mom>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D3Q19, double, double>(const StepArgs<double>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D3Q19, double, double>(const StepArgs<double>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D3Q19, double, double>(const StepArgs<double>&, int, int, cudaStream_t);
-template int launch_plain<D3Q19, float, __half>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D3Q19, float, __half>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D3Q19, float, __half>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D3Q19, float, __nv_bfloat16>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D3Q19, float, __nv_bfloat16>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D3Q19, float, __nv_bfloat16>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D2Q9, float, float>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D2Q9, float, float>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D2Q9, float, float>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D2Q9, double, double>(const StepArgs<double>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D2Q9, double, double>(const StepArgs<double>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D2Q9, double, double>(const StepArgs<double>&, int, int, cudaStream_t);
-template int launch_plain<D2Q9, float, __half>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D2Q9, float, __half>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D2Q9, float, __half>(const StepArgs<float>&, int, int, cudaStream_t);
-template int launch_plain<D2Q9, float, __nv_bfloat16>(const StepArgs<float>&, const Region&, const Region&, cudaStream_t, bool);
+template int launch_plain<D2Q9, float, __nv_bfloat16>(const StepArgs<float>&, const Region&, const Region&, const Region&, cudaStream_t, bool);
 template int launch_init<D2Q9, float, __nv_bfloat16>(const StepArgs<float>&, int, int, cudaStream_t);
 
 }  // namespace cglbm
