@@ -294,13 +294,16 @@ Region stream_region(const Region& R, int nx, int ny, int nz) { return grow(R, R
 // box around the nozzle wall at steps n0 and n0 + 1 (the step that n0 + 1
 // completes). Sites of margin around the wall: a bulk site's own pull and the
 // pulls of its neighbours (for their colour fractions) must see no wall node,
-// so it is at least three sites from one and two in the box suffice. 16-bit
-// storage keeps three: which kernel rounds a site decides its last bits.
+// so it is at least three sites from one and two in the box suffice. On plane 0
+// it also sees the substrate's ghost plane, a mean over densities one site
+// further out (Eq. 18), which pull from plane 1: where that is a wall plane
+// (gap 1) the box keeps three sites. So does 16-bit storage at any gap: which
+// kernel rounds a site decides its last bits.
 template <typename real>
 Region nozzle_box(const lbm_handle* h, const StepArgs<real>& p, long long n0) {
     const int nx = h->cfg.nx, ny = h->cfg.ny, nz = h->cfg.nz;
     if (!p.nozzle) return Region{0, 0, 0, 0, 0, 0};
-    const int margin = h->psize == 2 ? 3 : 2;
+    const int margin = h->psize == 2 || h->geom.gap == 1 ? 3 : 2;
     const long long ro = q20(h->geom.r_inner + h->geom.wall_thickness);
     const long long fx = (long long)kFx;
     const lbm_geometry& g = h->geom;
