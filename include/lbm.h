@@ -115,8 +115,8 @@ typedef struct {
     double nu0, nu_inf, lambda, n;  /* Cross: nu = nu_inf + (nu0 - nu_inf)/(1 + (lambda gdot)^n) */
     double K;              /* power law: nu = K gdot^(n-1) */
     double tau_min, tau_max;        /* clamps of the ink and mixture relaxation times */
-    double tol;            /* relative tolerance of the shear-rate iteration (<= 0: default) */
-    int max_iter;          /* iteration cap (<= 0: default 60) */
+    double tol;            /* relative tolerance of the shear-rate iteration (<= 0: default), an upper bound */
+    int max_iter;          /* cap on the iteration's steps (<= 0: default 60) */
 } lbm_rheology;
 
 /* Diagnostics, accumulated in FP64 on the device. */
