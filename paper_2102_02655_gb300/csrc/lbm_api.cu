@@ -141,12 +141,14 @@ bool unit_ratio(const lbm_config& c) {
 
 // The lattice's state is kept as 14 numbers per site (see PostState) instead
 // of 38 populations: FP32 at density ratio one on the fused path, and on
-// lattices periodic in z, which only that kernel fuses. Fixed from one
-// lbm_set_geometry to the next, which writes the state anew.
+// lattices periodic in z, which only that kernel fuses, up to the tile rows that
+// a launch holds (the phase-by-phase kernels, which those had, take any number).
+// Fixed from one lbm_set_geometry to the next, which writes the state anew.
 bool is_state(const lbm_handle* h) {
     if (h->cfg.storage != LBM_F32 || !unit_ratio(h->cfg) || h->cfg.velset != LBM_D3Q19) return false;
     if (h->cfg.path == LBM_PATH_PLAIN || 38.0 * (double)h->N >= 2147483647.0) return false;
-    return h->geom.z_mode == LBM_Z_PERIODIC || is_fused(h);
+    if (h->geom.z_mode == LBM_Z_PERIODIC) return (h->cfg.ny + kFusedTileH - 1) / kFusedTileH <= 65535;
+    return is_fused(h);
 }
 
 template <typename real>
