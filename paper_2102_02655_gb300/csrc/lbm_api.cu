@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <thread>
 #include <type_traits>
@@ -214,6 +215,7 @@ void fill_model(const lbm_handle* h, StepArgs<real>& p) {
     const double tol_default = sizeof(real) == 8 ? 1e-14 : 1e-6;
     p.tol = (real)(r.tol > 0 ? std::max(r.tol, tol_default) : tol_default);
     p.max_iter = r.max_iter > 0 ? r.max_iter : 60;
+    p.solve_lo = p.max_iter >= kSolveSteps ? real(1e-30) : std::numeric_limits<real>::infinity();
 }
 
 // geometry of step n-1 (index 0) and step n (index 1)
