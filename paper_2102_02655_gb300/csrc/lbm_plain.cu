@@ -119,12 +119,12 @@ __device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, con
     double bc0 = 0, bc1 = 0, de0 = 0, de1 = 0;
     int x, y, z;
     const bool site = region_site(Rs, p.nx, p.ny, &x, &y, &z) && !solid_at(p, x, y, z, 0);
-    // a warp takes one of the two forms (the boundary one serves plain sites too)
-    const bool plain = __all_sync(0xffffffffu, !site || plain_site(p, x, y, z));
+    const unsigned lanes = __ballot_sync(0xffffffffu, site);
     if (site) {
         real f[2][VS::Q];
         real bc[2] = {real(0), real(0)};
-        if (plain) pull_plain<VS, S>(p, x, y, z, f);
+        // a warp takes one of the two forms: the boundary one serves plain sites too
+        if (__all_sync(lanes, plain_site(p, x, y, z))) pull_plain<VS, S>(p, x, y, z, f);
         else pull_boundary<VS, S>(p, x, y, z, f, bc);
         real rY = 0, sd = 0;
 #pragma unroll
