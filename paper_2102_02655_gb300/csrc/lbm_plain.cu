@@ -112,8 +112,9 @@ __device__ __forceinline__ void post_put(const StepArgs<real>& p, long long s, c
     }
 }
 
-// 1. stream + densities (post-streaming) of every fluid node of step n-1 in Rs
-template <class VS, typename real, typename S>
+// 1. stream + densities (post-streaming) of every fluid node of step n-1 in Rs;
+//    kPlain: every site of Rs is plain (see plain_site)
+template <class VS, typename real, typename S, bool kPlain>
 __device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, const Region& Rs, const Region& R) {
     const long long comp = p.N + 2 * p.plane;
     double bc0 = 0, bc1 = 0, de0 = 0, de1 = 0;
@@ -123,9 +124,13 @@ __device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, con
     if (site) {
         real f[2][VS::Q];
         real bc[2] = {real(0), real(0)};
-        // a warp takes one of the two forms: the boundary one serves plain sites too
-        if (__all_sync(lanes, plain_site(p, x, y, z))) pull_plain<VS, S>(p, x, y, z, f);
-        else pull_boundary<VS, S>(p, x, y, z, f, bc);
+        if constexpr (kPlain) {
+            pull_plain<VS, S>(p, x, y, z, f);
+        } else {
+            // a warp takes one of the two forms: the boundary one serves plain sites too
+            if (__all_sync(lanes, plain_site(p, x, y, z))) pull_plain<VS, S>(p, x, y, z, f);
+            else pull_boundary<VS, S>(p, x, y, z, f, bc);
+        }
         real rY = 0, sd = 0;
 #pragma unroll
         for (int i = 0; i < VS::Q; ++i) { rY += f[0][i]; sd += f[1][i]; }
@@ -151,9 +156,10 @@ __device__ __forceinline__ void stream_density_body(const StepArgs<real>& p, con
     warp_add(p.acc + kAccDestroyed + 1, de1);
 }
 
-template <class VS, typename real, typename S>
-__global__ void __launch_bounds__(kThreads, 2) k_stream_density(StepArgs<real> p, Region Rs, Region R) {
-    stream_density_body<VS, real, S>(p, Rs, R);
+// (16-bit storage: 102 registers at most, so that five blocks fit an SM)
+template <class VS, typename real, typename S, bool kPlain>
+__global__ void __launch_bounds__(kThreads, Stored<S>::kDev ? 5 : 2) k_stream_density(StepArgs<real> p, Region Rs, Region R) {
+    stream_density_body<VS, real, S, kPlain>(p, Rs, R);
 }
 
 // The same with four threads to a site, one warp of the block for every fourth
@@ -665,11 +671,51 @@ template int launch_prev_from_f<D3Q19, double>(const StepArgs<double>&, double*,
 template int launch_prev_from_f<D2Q9, float>(const StepArgs<float>&, float*, float*, cudaStream_t);
 template int launch_prev_from_f<D2Q9, double>(const StepArgs<double>&, double*, double*, cudaStream_t);
 
-// Four threads to a site where the region is about one wave of the one-thread
-// form (the nozzle box; 64x32x32 whole: 21 -> 18 us). A larger region has the
-// warps to hide a thread's latency (880x240 FP64: 65 us against 76 split).
-inline bool split_stream(long long sites, bool state) {
-    return state || sites <= 150000;
+// Phase 1 over Rs; returns the number of kernels launched. Where no site has a
+// link from the nozzle or the top, the form without their rules: 72 registers
+// instead of 110 and seven blocks per SM instead of four. Periodic lattices take
+// it, and without a nozzle the planes below the top of any lattice larger than
+// one wave of the form with the rules (the top plane then has its own launch).
+// Four threads to a site where the other form has too few warps, up to 100,000
+// sites (40,000 in 2D, 19,456 - a block per SM - in periodic 16-bit lattices):
+// us per step of the phase-by-phase path, four threads / one,
+//   print run FP16  52k 54 / 54, 84k 62 / 64, 100k 67 / 67, 129k 78 / 74; FP32 33k 34 / 40, 84k 48 / 50, 129k 59 / 55;
+//   FP64  33k 112 / 121, 84k 222 / 227, 129k 278 / 278; 2D FP16  22k 37 / 41, 39k 42 / 43, 54k 46 / 42;
+//   periodic FP16  14k 29 / 31, 33k 33 / 33, 84k 49 / 38, 1.6M 569 / 397; FP32 14k 19 / 17; FP64 33k 72 / 68;
+//   lid FP16 (one thread, the top plane apart)  68k 44 / 44, 84k 49 / 48, 1.6M 575 / 408; FP64 84k 210 / 207;
+// and in a box beside the bulk kernel up to 150,000 (whole step, FP16 256x128x128,
+// 122k 343 / 347, 188k 370 / 369; 512x128x128, 188k 610 / 603; FP64 188k 5,852 / 6,029).
+// (With the rules in every one-thread kernel and four threads up to 150,000
+// sites: periodic FP16 84k 49, 1.6M 511; lid FP16 1.6M 522; print FP16 1.6M 514, now 478.)
+template <class VS, typename real, typename S>
+int launch_stream(const StepArgs<real>& p, const Region& Rs, const Region& R, cudaStream_t st) {
+    const long long sites = region_sites(Rs);
+    const bool periodic = p.z_mode == kZPeriodic;
+    auto four = [&](const Region& A) {
+        const long long cols = (long long)A.wx * A.wy;
+        k_stream_density_split<VS, real, S>
+            <<<dim3((unsigned)((cols + 31) / 32), (unsigned)(A.z1 - A.z0)), kThreads, 0, st>>>(p, A, R);
+    };
+    if constexpr (std::is_same<S, Mom>::value) {
+        four(Rs);
+        return 1;
+    } else {
+        constexpr long long sms = 152, wave = sms * 4 * kThreads;
+        if (periodic && !(Stored<S>::kDev && sites <= sms * kThreads)) {
+            k_stream_density<VS, real, S, true><<<region_grid(Rs), kThreads, 0, st>>>(p, Rs, R);
+        } else if (!periodic && !p.nozzle && sites > wave && p.nz > 1) {
+            Region below = Rs, top = Rs;
+            below.z1 = top.z0 = p.nz - 1;
+            k_stream_density<VS, real, S, true><<<region_grid(below), kThreads, 0, st>>>(p, below, R);
+            four(top);
+            return 2;
+        } else if (sites <= (region_sites(R) < p.N ? 150000 : (VS::kPlanar ? 40000 : 100000))) {
+            four(Rs);
+        } else {
+            k_stream_density<VS, real, S, false><<<region_grid(Rs), kThreads, 0, st>>>(p, Rs, R);
+        }
+        return 1;
+    }
 }
 
 template <class VS, typename real, typename S>
@@ -682,14 +728,7 @@ int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, con
         k_geo<real><<<geo_grid(G), kThreads, 0, st>>>(p, G);
         n = 1;
     }
-    if (split_stream(region_sites(Rs), std::is_same<S, Mom>::value)) {
-        const long long cols = (long long)Rs.wx * Rs.wy;
-        k_stream_density_split<VS, real, S>
-            <<<dim3((unsigned)((cols + 31) / 32), (unsigned)(Rs.z1 - Rs.z0)), kThreads, 0, st>>>(p, Rs, R);
-    } else {
-        if constexpr (!std::is_same<S, Mom>::value)
-            k_stream_density<VS, real, S><<<region_grid(Rs), kThreads, 0, st>>>(p, Rs, R);
-    }
+    n += launch_stream<VS, real, S>(p, Rs, R, st);
     if (p.nozzle) {
         k_created<VS, real, S><<<region_grid(R1), kThreads, 0, st>>>(p, R1, R);
         ++n;
@@ -706,7 +745,7 @@ int launch_plain(const StepArgs<real>& p, const Region& R, const Region& R1, con
         if (p.unit) k_collide<VS, real, true, S><<<region_grid(R), kThreads, 0, st>>>(p, R);
         else k_collide<VS, real, false, S><<<region_grid(R), kThreads, 0, st>>>(p, R);
     }
-    return 3 + n;
+    return 2 + n;
 }
 
 template <class VS, typename real, typename S>
