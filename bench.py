@@ -146,7 +146,8 @@ def _fused_source_sha():
 
 
 def _traffic_per_site():
-    """DRAM bytes per site update of the fused kernel from the committed ncu
+    """DRAM bytes per site update of the FP32 fused kernel over populations
+    (density ratio one has the state kernel since) from the committed ncu
     summary, if it was taken on the current kernel source."""
     try:
         with open(os.path.join(ROOT, "profiles", "k_fused_print_traffic.json")) as f:

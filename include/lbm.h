@@ -61,8 +61,9 @@ typedef enum { LBM_F64 = 0, LBM_F32 = 1, LBM_F16DEV = 2, LBM_BF16DEV = 3 } lbm_s
  * phase-by-phase kernels only in a box around the nozzle (D3Q19 only).
  * AUTO picks FUSED where it applies. Both give the same result. Off the PLAIN
  * path an FP32 D3Q19 lattice of density ratio one (with a substrate and an open
- * top, or periodic in z) keeps its state in the population buffers as the 14
- * numbers a regularised collision leaves, FP32 as the populations. */
+ * top, or periodic in z with ny <= 524,280) keeps its state in the population
+ * buffers as the 14 numbers a regularised collision leaves, FP32 as the
+ * populations. */
 typedef enum { LBM_PATH_AUTO = 0, LBM_PATH_PLAIN = 1, LBM_PATH_FUSED = 2 } lbm_path;
 
 typedef enum { LBM_Z_PERIODIC = 0, LBM_Z_WALLS = 1 } lbm_zmode;
